@@ -40,6 +40,18 @@ constexpr int kDvrGrad = 1;  // the same, keeping transmittance checkpoints for 
 constexpr int kMop = 2;      // maximum-opacity projection (Sec. V-A, Table I)
 constexpr int kMip = 3;      // maximum-intensity projection
 
+// Resident CTAs per SM that a k_render variant's registers are allotted for (the persistent grid is
+// this many per SM).  The batch's corner words bound them: a sample holds 2 (u8), 4 (16-bit) or 8
+// (f32, compact slots) words until its interpolation, beside its weights.  At 5 CTAs (96
+// registers) the variants with 8 words spill; emission/absorption on 16-bit slots is faster with
+// 8 samples at 4 CTAs than with 6 at 5, the projections (longer rays, no tail of terminated ones)
+// and u8 are not.  general: the level-scaled and sparse-table variants (one sample at a time).
+__host__ __device__ constexpr int render_ctas(int dt, bool quad, int mode, bool general) {
+    if (general) return 5;
+    if (!quad || dt == VOL_F32) return 4;
+    return dt != VOL_U8 && mode != kMop && mode != kMip ? 4 : 5;
+}
+
 // Counter words of one render (device memory, reset before each pass).
 enum Counter : int {
     kWork = 0,       // next work item (tile or suspended-ray chunk)
@@ -97,6 +109,7 @@ struct VolDev {
     int nlevels;
     const uint32_t* pt;            // flat page table, or the sparse table's pool
     int sparse;                    // 1: three-level sparse page table
+    int wide;                      // 1: an axis is longer than 2^23 voxels
     const float2* range;           // per slot: min and max stored value (stored units)
     // per slot: the TF-entry span of each macro-cell (8 x 8 x 8 cells per brick, or B per axis
     // when B < 8; cell c covers local voxels [c M, c M + M] per axis, M = B >> cbits): byte 0 the
@@ -118,6 +131,7 @@ struct RenderDev {
     int refill_thresh;  // refill lanes when fewer than this many are active
     const float4* tf;
     float step, et;
+    float neg_zero;     // -0.0f (render_common.cuh: packed products)
     float4 bg;
     int lod_mode, lod_bias;
     int skip_empty;     // empty-space skipping: launch the ES variant of the kernel
@@ -196,7 +210,6 @@ struct TraceDev {
 cudaError_t launch_render(int dtype, int mode, const RenderDev& p, int grid, cudaStream_t s);
 cudaError_t launch_backward(int dtype, const BackwardDev& p, int grid, cudaStream_t s);
 cudaError_t launch_trace(const TraceDev& p, cudaStream_t s);
-int render_blocks_per_sm(int dtype, bool grad);
 // Maximum projections (kernels_project.cu): the k_render variant for mode kMop or kMip.
 const void* pick_render_projection(int dtype, int brick, bool quad, bool lod, int mode);
 // Level-scaled sampling (kernels_lstep.cu): the emission/absorption variant.

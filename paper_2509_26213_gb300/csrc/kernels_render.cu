@@ -545,13 +545,6 @@ cudaError_t launch_trace(const TraceDev& p, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-int render_blocks_per_sm(int dtype, bool grad) {
-    int n = 0;
-    const void* fn = pick_render(dtype, 64, true, false, grad);
-    if (!fn || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kRenderThreads, 0) != cudaSuccess) return 1;
-    return n > 0 ? n : 1;
-}
-
 int backward_blocks_per_sm(int dtype, bool lod, bool tape) {
     int n = 0;
     const void* fn = pick_backward(dtype, lod, tape);

@@ -272,7 +272,6 @@ struct vol_s {
     int64_t allocations = 0;  // device and pinned-host allocations since vol_create
     bool counters_collected = true;  // the counter words hold a pass collect_pass already read
     unsigned* last_counters = nullptr;  // the counter words of the last pass (NULL: counters)
-    int occ_cache[4][2] = {{0}};
     ViewDev noalloc_views[VOL_NOALLOC_MAX_VIEWS];  // vol_render_noalloc's host staging of its view table
 };
 
@@ -336,6 +335,7 @@ VolDev vol_dev(const vol_t v) {
     }
     for (int a = 0; a < 3; ++a) d.D0f[a] = (float)v->lay.dims[a];
     d.sparse = v->sparse ? 1 : 0;
+    for (int a = 0; a < 3; ++a) d.wide |= v->lay.dims[a] > (1 << 23);
     return d;
 }
 
@@ -570,11 +570,17 @@ bool all_resident(const vol_t v, bool lod) {
     return true;
 }
 
-int grid_for(vol_t v, int dtype, bool grad, int ctas_per_sm) {
-    int& occ = v->occ_cache[dtype][grad ? 1 : 0];
-    if (!occ) occ = render_blocks_per_sm(dtype, grad);
-    int per = ctas_per_sm > 0 ? std::min(ctas_per_sm, occ) : occ;
-    return std::max(1, per * v->nsm);
+int render_mode(const vol_params& p, bool grad) {
+    if (grad) return kDvrGrad;
+    if (p.composite == VOL_COMPOSITE_MOP) return kMop;
+    if (p.composite == VOL_COMPOSITE_MIP) return kMip;
+    return kDvr;
+}
+
+int grid_for(vol_t v, const vol_params& p, bool grad) {
+    const int occ = render_ctas(v->dtype, v->lay.layout == 0, render_mode(p, grad),
+                                v->sparse || (p.flags & VOL_RENDER_LEVEL_STEP) != 0);
+    return (p.ctas_per_sm > 0 ? std::min(p.ctas_per_sm, occ) : occ) * v->nsm;
 }
 
 int ensure_miss_buffers(vol_t v) {
@@ -600,16 +606,10 @@ int ensure_miss_buffers(vol_t v) {
     return VOL_OK;
 }
 
-int render_mode(const vol_params& p, bool grad) {
-    if (grad) return kDvrGrad;
-    if (p.composite == VOL_COMPOSITE_MOP) return kMop;
-    if (p.composite == VOL_COMPOSITE_MIP) return kMip;
-    return kDvr;
-}
-
 RenderDev render_args(vol_t v) {
     RenderDev p{};
     p.vol = vol_dev(v);
+    p.neg_zero = -0.0f;
     p.views = v->views_dev;
     p.nviews = v->nviews;
     p.tile_w = v->params.tile_w;
@@ -724,7 +724,7 @@ int run_pass(vol_t v, bool resume, bool may_miss) {
     CK(v, cudaMemsetAsync(v->counters, 0, sizeof(unsigned) * kNumCounters, v->stream));
     v->counters_collected = false;
     v->last_counters = v->counters;
-    const int grid = grid_for(v, v->dtype, v->grad, v->params.ctas_per_sm);
+    const int grid = grid_for(v, v->params, v->grad);
     if (v->ev_pass_start) CK(v, cudaEventRecord(v->ev_pass_start, v->stream));
     CK(v, launch_render(v->dtype, render_mode(v->params, v->grad), p, grid, v->stream));
     if (v->ev_pass_end) CK(v, cudaEventRecord(v->ev_pass_end, v->stream));
@@ -2053,6 +2053,7 @@ extern "C" int vol_render_noalloc(vol_t v, const vol_camera* cams, int nviews, c
     CK(v, cudaMemsetAsync(counters, 0, sizeof(unsigned) * kNumCounters, v->stream));
 
     RenderDev r{};
+    r.neg_zero = -0.0f;
     r.vol = vol_dev(v);
     r.views = views_dev;
     r.nviews = nviews;
@@ -2073,7 +2074,7 @@ extern "C" int vol_render_noalloc(vol_t v, const vol_camera* cams, int nviews, c
     r.nsamp = nsamples_dev;
     r.counters = counters;
     r.nrays = rays;  // no request table, no suspension buffers, no usage stamps, no checkpoints
-    const int grid = grid_for(v, v->dtype, false, p.ctas_per_sm);
+    const int grid = grid_for(v, p, false);
     // the per-render counters describe this call, as they do after vol_render (the state a
     // gradient render left for vol_render_backward is not touched)
     v->stats = vol_stats{};
