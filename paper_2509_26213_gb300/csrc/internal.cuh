@@ -226,24 +226,21 @@ cudaError_t launch_tile_order(int* cost, int* order, int ntiles, int* buckets, c
 int backward_blocks_per_sm(int dtype, bool lod, bool tape);
 
 // ---- launchers (kernels_volume.cu) ----
-// Write every brick of a dense level (src of src_dtype) into atlas slots.
-cudaError_t launch_upload_level(int dst_dtype, int src_dtype, const void* src, const VolDev& vol,
-                                int level, const uint32_t* slots_of_bricks, long long nbricks,
-                                cudaStream_t s);
-// Write n packed (B+1)^3 bricks (src of src_dtype, device) into slots[i] (device array).
-cudaError_t launch_upload_bricks(int dst_dtype, int src_dtype, const void* src, const VolDev& vol,
-                                 const uint32_t* slots, long long n, cudaStream_t s);
+// Each of these fills whole slots: the voxels, range[slot] = (min, max) of the stored values and
+// the slot's macro-cell TF-entry spans in cells (NULL: none).
+// Every brick of a dense level (src of src_dtype).
+cudaError_t launch_upload_level(int dst_dtype, int src_dtype, const void* src, const VolDev& vol, int level, float2* range,
+                                uint16_t* cells, const uint32_t* slots_of_bricks, long long nbricks, cudaStream_t s);
+// n packed (B+1)^3 bricks (src of src_dtype, device-accessible) into slots[i] (device array).
+cudaError_t launch_upload_bricks(int dst_dtype, int src_dtype, const void* src, const VolDev& vol, float2* range,
+                                 uint16_t* cells, const uint32_t* slots, long long n, cudaStream_t s);
 // Build level `level` (all bricks; slots_of_bricks indexed by brick id) from level-1.
-cudaError_t launch_downsample(int dtype, const VolDev& vol, int level, const uint32_t* slots_of_bricks,
-                              long long nbricks, unsigned* err, cudaStream_t s);
+cudaError_t launch_downsample(int dtype, const VolDev& vol, int level, float2* range, uint16_t* cells,
+                              const uint32_t* slots_of_bricks, long long nbricks, unsigned* err, cudaStream_t s);
 // Adjoint of one box-filter level: fine[i] += coarse[parent(i)] * (shares of i) / 8, for the
 // level of dims Dfine filtered into the level of coarse (a child index past the edge counts as
 // the last voxel, as in the filter).
 cudaError_t launch_downsample_transpose(const float* coarse, float* fine, const int Dfine[3], cudaStream_t s);
-// range[slots[i]] = (min, max) of the stored values of each listed slot, and the slot's macro-cell
-// TF-entry spans in cells (one CTA per slot).
-cudaError_t launch_slot_range(int dtype, const VolDev& vol, float2* range, uint16_t* cells, const uint32_t* slots,
-                              long long n, cudaStream_t s);
 // pt[idx[i]] = val[i] for i < n (atomic exchange; Sec. III-E parallel insert/remove).
 cudaError_t launch_pt_update(uint32_t* pt, const uint32_t* idx, const uint32_t* val, int n,
                              cudaStream_t s);

@@ -852,10 +852,9 @@ int load_requests(vol_t v) {
         v->stats.bytes_loaded += (int64_t)(n * src_bytes);
         CK(v, cudaMemcpyAsync(v->stage_dev, v->stage_host, src_bytes * n, cudaMemcpyHostToDevice, v->stream));
         CK(v, cudaMemcpyAsync(v->stage_slots_dev, slots.data(), sizeof(uint32_t) * n, cudaMemcpyHostToDevice, v->stream));
-        CK(v, launch_upload_bricks(v->dtype, v->prov_dtype, v->stage_dev, vol_dev(v), v->stage_slots_dev, (long long)n,
-                                   v->stream));
-        CK(v, launch_slot_range(v->dtype, vol_dev(v), v->range, v->cells, v->stage_slots_dev, (long long)n, v->stream));
-        v->stats.launches += 2;
+        CK(v, launch_upload_bricks(v->dtype, v->prov_dtype, v->stage_dev, vol_dev(v), v->range, v->cells, v->stage_slots_dev,
+                                   (long long)n, v->stream));
+        v->stats.launches += 1;
         if (int rc = flush_pt_updates(v)) return rc;
         CK(v, cudaStreamSynchronize(v->stream));  // the pinned stage is reused by the next batch
     }
@@ -1111,11 +1110,10 @@ int ovl_publish(vol_t v, int* published) {
     auto& R = v->ring;
     const int n = J.n, st = J.start;
     const size_t bb = R.brick_bytes;
-    CK(v, launch_upload_bricks(v->dtype, v->prov_dtype, R.host_dev + (size_t)st * bb, vol_dev(v), R.slots_dev + st,
-                               (long long)n, v->stream));
-    CK(v, launch_slot_range(v->dtype, vol_dev(v), v->range, v->cells, R.slots_dev + st, (long long)n, v->stream));
+    CK(v, launch_upload_bricks(v->dtype, v->prov_dtype, R.host_dev + (size_t)st * bb, vol_dev(v), v->range, v->cells,
+                               R.slots_dev + st, (long long)n, v->stream));
     CK(v, launch_pt_update(v->pt, R.ptis_dev + st, R.slots_dev + st, n, v->stream));
-    v->stats.launches += 3;
+    v->stats.launches += 2;
     cudaEvent_t ev = nullptr;
     if (!R.spare.empty()) {
         ev = R.spare.back();
@@ -1397,28 +1395,29 @@ int vol_upload_level(vol_t v, int level, const void* src, int src_dtype, int src
     const int64_t nb = level_nbricks(v, level);
     if (nb > v->lay.nslots) return fail(v, VOL_ERR_CACHE_FULL, "level does not fit the brick cache");
     ++v->op_epoch;
-    std::vector<uint32_t> slots((size_t)nb);
+    const uint32_t off = (uint32_t)v->lay.level_pt_offset[level];
+    uint32_t slot;
     for (int64_t b = 0; b < nb; ++b)
-        if (int rc = slot_for(v, (uint32_t)(v->lay.level_pt_offset[level] + b), &slots[(size_t)b])) return rc;
+        if (int rc = slot_for(v, off + (uint32_t)b, &slot)) return rc;
     const int64_t nvox = v->lay.level_dims[level][0] * v->lay.level_dims[level][1] * v->lay.level_dims[level][2];
     const size_t sbytes = (size_t)nvox * bpv_of(src_dtype);
     const void* dsrc = src;
     void* tmp = nullptr;
-    uint32_t* dslots = nullptr;
-    CK(v, dev_alloc(v, (void**)&dslots, sizeof(uint32_t) * (size_t)nb));
     if (!src_on_device) {
         cudaError_t e = dev_alloc(v, (void**)&tmp, sbytes);
-        if (e != cudaSuccess) { cudaFree(dslots); return cuda_fail(v, e, "upload staging"); }
+        if (e != cudaSuccess) return cuda_fail(v, e, "upload staging");
         e = cudaMemcpyAsync(tmp, src, sbytes, cudaMemcpyHostToDevice, v->stream);
-        if (e != cudaSuccess) { cudaFree(dslots); cudaFree(tmp); return cuda_fail(v, e, "upload copy"); }
+        if (e != cudaSuccess) { cudaFree(tmp); return cuda_fail(v, e, "upload copy"); }
         dsrc = tmp;
     }
-    cudaError_t e = cudaMemcpyAsync(dslots, slots.data(), sizeof(uint32_t) * (size_t)nb, cudaMemcpyHostToDevice, v->stream);
-    if (e == cudaSuccess) e = launch_upload_level(v->dtype, src_dtype, dsrc, vol_dev(v), level, dslots, nb, v->stream);
-    if (e == cudaSuccess) e = launch_slot_range(v->dtype, vol_dev(v), v->range, v->cells, dslots, nb, v->stream);
-    int rc = e == cudaSuccess ? flush_pt_updates(v) : cuda_fail(v, e, "upload_level kernel");
-    cudaError_t e2 = cudaStreamSynchronize(v->stream);
-    cudaFree(dslots);
+    // the level's slots are its entries of the device page table, current once the updates are queued
+    int rc = flush_pt_updates(v);
+    if (!rc) {
+        const cudaError_t e = launch_upload_level(v->dtype, src_dtype, dsrc, vol_dev(v), level, v->range, v->cells, v->pt + off,
+                                                  nb, v->stream);
+        if (e != cudaSuccess) rc = cuda_fail(v, e, "upload_level kernel");
+    }
+    const cudaError_t e2 = cudaStreamSynchronize(v->stream);
     if (tmp) cudaFree(tmp);
     if (rc) return rc;
     if (e2 != cudaSuccess) return cuda_fail(v, e2, "upload_level");
@@ -1443,9 +1442,8 @@ int vol_upload_brick(vol_t v, int level, const int32_t brick[3], const void* src
         dsrc = v->stage_dev;
     }
     CK(v, cudaMemcpyAsync(v->stage_slots_dev, &s, sizeof(uint32_t), cudaMemcpyHostToDevice, v->stream));
-    CK(v, launch_upload_bricks(v->dtype, src_dtype, dsrc, vol_dev(v), v->stage_slots_dev, 1, v->stream));
-    CK(v, launch_slot_range(v->dtype, vol_dev(v), v->range, v->cells, v->stage_slots_dev, 1, v->stream));
-    v->stats.launches += 2;
+    CK(v, launch_upload_bricks(v->dtype, src_dtype, dsrc, vol_dev(v), v->range, v->cells, v->stage_slots_dev, 1, v->stream));
+    v->stats.launches += 1;
     if (int rc = flush_pt_updates(v)) return rc;
     CK(v, cudaStreamSynchronize(v->stream));
     return VOL_OK;
@@ -1466,24 +1464,16 @@ int vol_build_lod(vol_t v, int from_level) {
         // keep the source level while allocating the coarse one
         for (int64_t b = 0; b < level_nbricks(v, l - 1); ++b)
             v->protect[v->pt_host[(size_t)(v->lay.level_pt_offset[l - 1] + b)]] = v->op_epoch;
-        std::vector<uint32_t> slots((size_t)nb);
+        const uint32_t off = (uint32_t)v->lay.level_pt_offset[l];
+        uint32_t slot;
         for (int64_t b = 0; b < nb; ++b)
-            if (int rc = slot_for(v, (uint32_t)(v->lay.level_pt_offset[l] + b), &slots[(size_t)b])) return rc;
-        uint32_t* dslots = nullptr;
-        CK(v, dev_alloc(v, (void**)&dslots, sizeof(uint32_t) * (size_t)nb));
-        cudaError_t e = cudaMemcpyAsync(dslots, slots.data(), sizeof(uint32_t) * (size_t)nb, cudaMemcpyHostToDevice, v->stream);
-        int rc = VOL_OK;
-        if (e == cudaSuccess) rc = flush_pt_updates(v);  // the source level's entries must be live
-        if (e == cudaSuccess && !rc) e = launch_downsample(v->dtype, vol_dev(v), l, dslots, nb, v->aux, v->stream);
-        if (e == cudaSuccess && !rc) e = launch_slot_range(v->dtype, vol_dev(v), v->range, v->cells, dslots, nb, v->stream);
-        cudaError_t e2 = cudaStreamSynchronize(v->stream);
-        cudaFree(dslots);
-        if (rc) return rc;
-        if (e != cudaSuccess) return cuda_fail(v, e, "downsample");
-        if (e2 != cudaSuccess) return cuda_fail(v, e2, "downsample");
+            if (int rc = slot_for(v, off + (uint32_t)b, &slot)) return rc;
+        if (int rc = flush_pt_updates(v)) return rc;  // both levels' entries must be live
+        CK(v, launch_downsample(v->dtype, vol_dev(v), l, v->range, v->cells, v->pt + off, nb, v->aux, v->stream));
     }
     unsigned aux0 = 0;
-    CK(v, cudaMemcpy(&aux0, v->aux, sizeof(unsigned), cudaMemcpyDeviceToHost));
+    CK(v, cudaMemcpyAsync(&aux0, v->aux, sizeof(unsigned), cudaMemcpyDeviceToHost, v->stream));
+    CK(v, cudaStreamSynchronize(v->stream));
     if (aux0) return fail(v, VOL_ERR_DEVICE, "downsample met a non-resident brick");
     return VOL_OK;
 }

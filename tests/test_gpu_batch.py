@@ -66,7 +66,7 @@ def test_axis_longer_than_the_floor_constant(P, orc):
     rng = np.random.default_rng(3)
     raw = rng.integers(0, 256, D[::-1], dtype=np.uint8)
     tf = synth.tf_ramp(alpha_start=0.1, alpha_max=0.3)
-    params = {"step": 0.5, "et": 2.0, "lod_mode": 0}
+    params = {"step": 0.75, "et": 2.0, "lod_mode": 0}  # (below 2^24 samples on the diagonal)
     c = np.array([D[0] - 8.0, 1.5, 1.0])
     cam = synth.look_at(tuple(c + np.array([2.0, 9.0, 4.0])), tuple(c), 16, 12, fov_deg=60.0)
     vol = P.Volume(D, "u8", 4, 1)
