@@ -797,7 +797,10 @@ __device__ __forceinline__ void request_brick(const RenderDev& P, uint32_t key) 
     uint32_t h = hash_key(key) & P.req_cap_mask;
     int state = 2;  // 0 new, 1 present, 2 overflow
     for (int probe = 0; probe < kMaxProbe; ++probe) {
-        const uint32_t prev = atomicCAS(&P.req_table[h], 0u, key);
+        // (a plain read first: thousands of rays ask for the same few bricks, and additions to one
+        // address are serialised; a key once written stays)
+        uint32_t prev = __ldcg(&P.req_table[h]);
+        if (prev != key) prev = atomicCAS(&P.req_table[h], 0u, key);
         if (prev == 0u) { state = 0; break; }
         if (prev == key) { state = 1; break; }
         h = (h + 1) & P.req_cap_mask;
@@ -822,7 +825,8 @@ __device__ __forceinline__ void request_brick64(const RenderDev& P, unsigned lon
     uint32_t h = hash_key((uint32_t)key ^ hash_key((uint32_t)(key >> 32))) & P.req_cap_mask;
     int state = 2;  // 0 new, 1 present, 2 overflow
     for (int probe = 0; probe < kMaxProbe; ++probe) {
-        const unsigned long long prev = atomicCAS(&P.req_table64[h], 0ull, key);
+        unsigned long long prev = __ldcg(&P.req_table64[h]);
+        if (prev != key) prev = atomicCAS(&P.req_table64[h], 0ull, key);
         if (prev == 0ull) { state = 0; break; }
         if (prev == key) { state = 1; break; }
         h = (h + 1) & P.req_cap_mask;
