@@ -221,7 +221,8 @@ const void* pick_render_sparse(int dtype, int brick, bool quad, bool lod);
 const void* pick_render_skip(int dtype, int brick, bool quad, bool lod, int mode);
 const void* pick_render_skip_projection(int dtype, int brick, bool quad, bool lod, int mode);
 // order[] = tiles sorted by descending log2 bucket of cost[] (longest ray first); zeroes cost[].
-// buckets: 64 ints of device scratch.
+// buckets: 64 ints of device scratch.  Up to kOrderSmall tiles in one launch, else two.
+constexpr int kOrderSmall = 8192;
 cudaError_t launch_tile_order(int* cost, int* order, int ntiles, int* buckets, cudaStream_t s);
 int backward_blocks_per_sm(int dtype, bool lod, bool tape);
 

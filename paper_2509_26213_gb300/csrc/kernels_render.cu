@@ -408,6 +408,43 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_scatter(int* cost, int*
     }
 }
 
+// The same in one launch of one CTA, for a few tiles: the lanes of a warp on one bucket add to it
+// together.  Up to kOrderSmall tiles (a 512 x 512 view) that takes no longer than the two kernels
+// above, and their launches and the zeroing of the buckets go: what a small frame's time is made of.
+
+__global__ void __launch_bounds__(1024) k_order_small(int* cost, int* order, int ntiles) {
+    __shared__ int s_count[32], s_next[32];
+    if (threadIdx.x < 32) s_count[threadIdx.x] = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int i0 = 0; i0 < ntiles; i0 += 1024) {
+        const int i = i0 + (int)threadIdx.x;
+        const int b = i < ntiles ? cost_bucket(cost[i]) : -1;
+        const unsigned m = __match_any_sync(kFull, b);
+        if (b >= 0 && lane == __ffs(m) - 1) atomicAdd(&s_count[b], __popc(m));
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        int base = 0;
+        for (int q = 31; q > lane; --q) base += s_count[q];
+        s_next[lane] = base;
+    }
+    __syncthreads();
+    for (int i0 = 0; i0 < ntiles; i0 += 1024) {
+        const int i = i0 + (int)threadIdx.x;
+        const int b = i < ntiles ? cost_bucket(cost[i]) : -1;
+        const unsigned m = __match_any_sync(kFull, b);
+        const int leader = __ffs(m) - 1;
+        int base = 0;
+        if (b >= 0 && lane == leader) base = atomicAdd(&s_next[b], __popc(m));
+        base = __shfl_sync(kFull, base, leader);
+        if (b >= 0) {
+            order[base + __popc(m & ((1u << lane) - 1u))] = i;
+            cost[i] = 0;
+        }
+    }
+}
+
 // ------------------------------------------------------------------ trace
 
 __global__ void k_trace(const __grid_constant__ TraceDev P) {
@@ -531,6 +568,10 @@ cudaError_t launch_backward(int dtype, const BackwardDev& p, int grid, cudaStrea
 
 cudaError_t launch_tile_order(int* cost, int* order, int ntiles, int* buckets, cudaStream_t s) {
     if (ntiles <= 0) return cudaSuccess;
+    if (ntiles <= kOrderSmall) {
+        k_order_small<<<1, 1024, 0, s>>>(cost, order, ntiles);
+        return cudaGetLastError();
+    }
     cudaError_t e = cudaMemsetAsync(buckets, 0, sizeof(int) * 64, s);
     if (e != cudaSuccess) return e;
     const int grid = (ntiles + kOrderThreads - 1) / kOrderThreads;

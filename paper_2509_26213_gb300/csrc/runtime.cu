@@ -1773,7 +1773,7 @@ int vol_render(vol_t v, const vol_camera* cams, int nviews, const float* tf_dev,
     if (rc == VOL_OK && !preview) v->have_forward = true;
     if (rc == VOL_OK || rc == VOL_ERR_INCOMPLETE) {
         CK(v, launch_tile_order(v->tile_cost, v->tile_order, (int)tiles, v->order_buckets, v->stream));
-        v->stats.launches += 2;
+        v->stats.launches += tiles <= kOrderSmall ? 1 : 2;
         v->order_ready = true;
     }
     return rc;
