@@ -80,6 +80,7 @@ class Volume:
                                     ctypes.byref(h)))
         self.h = h
         self._provider = None
+        self._renders = 0  # vol_render calls
         lay = C.vol_layout()
         C.check(self.lib.vol_get_layout(self.h, ctypes.byref(lay)), self.h)
         self.layout = lay
@@ -198,6 +199,7 @@ class Volume:
             raise ValueError("out must be a contiguous float32 CUDA or pinned host tensor of sum(w*h) x 4")
         ns = torch.empty(npx, dtype=torch.int32, device=dev) if nsamples else None
         p = params_struct(**params, grad=grad)
+        self._renders += 1
         rc = self.lib.vol_render(self.h, arr, len(cams), ctypes.c_void_p(tf.data_ptr()), ctypes.byref(p),
                                  ctypes.c_void_p(out.data_ptr()),
                                  ctypes.c_void_p(ns.data_ptr() if ns is not None else 0))
@@ -270,14 +272,14 @@ class RaycastFn(torch.autograd.Function):
             volume.build_lod(0)
         out = volume.render(cams, tf.detach(), params, grad=True)
         ctx.volume = volume
-        ctx.frame = volume.stats()["frame"]
+        ctx.render = volume._renders  # (vol_get_stats would wait for the frame)
         ctx.shapes = (density.shape, tf.shape)
         return out
 
     @staticmethod
     def backward(ctx, grad_out):
         vol = ctx.volume
-        if vol.stats()["frame"] != ctx.frame:
+        if vol._renders != ctx.render:
             raise RuntimeError("the volume rendered again between forward and backward")
         dvox = torch.zeros(ctx.shapes[0], dtype=torch.float32, device=grad_out.device) if ctx.needs_input_grad[0] else None
         dtf = torch.zeros(ctx.shapes[1], dtype=torch.float32, device=grad_out.device) if ctx.needs_input_grad[1] else None
