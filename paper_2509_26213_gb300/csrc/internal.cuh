@@ -182,6 +182,8 @@ struct BackwardDev {
     float* dtf;
     float* dvox;                // level-0 gradient (NULL: none)
     float* dlev[kMaxLevels];    // gradient of each level's voxels; dlev[0] = dvox
+    float4* gq[kMaxLevels];     // gradient quads of each level (gq[0] NULL: add to dlev directly)
+    float4* dtf_tabs;           // 256 entries per warp of the grid, zeroed
     int lod_mode, lod_bias;
     unsigned* counters;
     const float* ckpt;
@@ -224,6 +226,11 @@ const void* pick_render_skip_projection(int dtype, int brick, bool quad, bool lo
 // buckets: 64 ints of device scratch.  Up to kOrderSmall tiles in one launch, else two.
 constexpr int kOrderSmall = 8192;
 cudaError_t launch_tile_order(int* cost, int* order, int ntiles, int* buckets, cudaStream_t s);
+// dvox += (add) or = the per-voxel sums of a level's gradient quads.
+cudaError_t launch_gather_quads(const float4* gq, float* dvox, const int D[3], bool add, cudaStream_t s);
+// dtf += the sum of n 256-entry tables.
+cudaError_t launch_sum_tables(const float4* tabs, int n, float* dtf, cudaStream_t s);
+int backward_warps_per_cta();
 int backward_blocks_per_sm(int dtype, bool lod, bool tape);
 
 // ---- launchers (kernels_volume.cu) ----

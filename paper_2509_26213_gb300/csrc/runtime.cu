@@ -204,6 +204,10 @@ struct vol_s {
     size_t ray_n_cap = 0;
     float* dlev_buf = nullptr;  // adjoint with LOD: gradients of levels 1..L-1
     size_t dlev_cap = 0;
+    float4* gq_buf = nullptr;   // adjoint: gradient quads of every level, and the warps' dL/dtf tables
+    size_t gq_cap = 0;
+    float4* dtf_tabs = nullptr;
+    size_t dtf_tabs_cap = 0;
 
     // provider
     vol_provider_fn prov = nullptr;
@@ -1330,7 +1334,7 @@ void vol_destroy(vol_t v) {
     else cudaDeviceSynchronize();
     void* bufs[] = {v->atlas, v->pt, v->last_used, v->counters, v->aux, v->upd_dev, v->views_dev, v->req_table,
                     v->req_list, v->susp[0], v->susp[1], v->ckpt, v->tape, v->ray_n, v->stage_dev, v->stage_slots_dev,
-                    v->tile_cost, v->tile_order, v->order_buckets, v->range, v->cells, v->dlev_buf, v->req_table64,
+                    v->tile_cost, v->tile_order, v->order_buckets, v->range, v->cells, v->dlev_buf, v->gq_buf, v->dtf_tabs, v->req_table64,
                     v->req_list64};
     for (void* b : bufs)
         if (b) cudaFree(b);
@@ -1838,11 +1842,43 @@ int vol_render_backward(vol_t v, const float* drgba_dev, float* dtf_dev, float* 
         for (int l = 1; l < v->L; ++l)
             tot += (size_t)(v->lay.level_dims[l][0] * v->lay.level_dims[l][1] * v->lay.level_dims[l][2]);
         if (int rc = ensure(v, v->dlev_buf, v->dlev_cap, tot, "level gradient buffers")) return rc;
-        CK(v, cudaMemsetAsync(v->dlev_buf, 0, sizeof(float) * tot, v->stream));
         size_t off = 0;
         for (int l = 1; l < v->L; ++l) {
             b.dlev[l] = v->dlev_buf + off;
             off += (size_t)(v->lay.level_dims[l][0] * v->lay.level_dims[l][1] * v->lay.level_dims[l][2]);
+        }
+    }
+    const int nlev = lod ? v->L : 1;
+    if (dvoxel_dev) {
+        // Gradient quads cost 16 B of zeroing, 16 B of reading and the voxel's own update per voxel,
+        // and save 6 of 8 reductions per cell visit: taken when the rays' samples (about an eighth of
+        // pixels x longest axis / step in the measured frames) outnumber the voxels, and the memory
+        // can be had.
+        size_t quads = 0, voxels = 0;
+        for (int l = 0; l < nlev; ++l) {
+            const int64_t* D = v->lay.level_dims[l];
+            voxels += (size_t)(D[0] * D[1] * D[2]);
+            quads += (size_t)(D[0] * D[1] * (D[2] + 1));
+        }
+        const double longest = (double)std::max({v->lay.dims[0], v->lay.dims[1], v->lay.dims[2]});
+        if ((double)v->nrays * longest / (double)v->params.step >= 8.0 * (double)voxels) {
+            if (ensure(v, v->gq_buf, v->gq_cap, quads, "gradient quads") == VOL_OK) {
+                CK(v, cudaMemsetAsync(v->gq_buf, 0, sizeof(float4) * quads, v->stream));
+                size_t off = 0;
+                for (int l = 0; l < nlev; ++l) {
+                    b.gq[l] = v->gq_buf + off;
+                    off += (size_t)(v->lay.level_dims[l][0] * v->lay.level_dims[l][1] * (v->lay.level_dims[l][2] + 1));
+                }
+            } else {
+                cudaGetLastError();  // (the failed allocation: the gradients go to the voxels directly)
+                v->err.clear();
+            }
+        }
+        if (lod && !b.gq[0]) {
+            size_t tot = 0;
+            for (int l = 1; l < v->L; ++l)
+                tot += (size_t)(v->lay.level_dims[l][0] * v->lay.level_dims[l][1] * v->lay.level_dims[l][2]);
+            CK(v, cudaMemsetAsync(v->dlev_buf, 0, sizeof(float) * tot, v->stream));
         }
     }
     b.counters = v->counters;
@@ -1857,8 +1893,24 @@ int vol_render_backward(vol_t v, const float* drgba_dev, float* dtf_dev, float* 
     v->counters_collected = false;  // vol_get_stats adds the adjoint's device-side check count
     v->last_counters = v->counters;
     const int grid = backward_blocks_per_sm(v->dtype, lod, b.tape != nullptr) * v->nsm;
+    if (dtf_dev) {
+        const size_t n = (size_t)grid * backward_warps_per_cta() * 256;
+        if (int rc = ensure(v, v->dtf_tabs, v->dtf_tabs_cap, n, "dL/dtf tables")) return rc;
+        CK(v, cudaMemsetAsync(v->dtf_tabs, 0, sizeof(float4) * n, v->stream));
+        b.dtf_tabs = v->dtf_tabs;
+    }
     CK(v, launch_backward(v->dtype, b, grid, v->stream));
     v->stats.launches += 1;
+    if (dtf_dev) {
+        CK(v, launch_sum_tables(v->dtf_tabs, grid * backward_warps_per_cta(), dtf_dev, v->stream));
+        v->stats.launches += 1;
+    }
+    if (b.gq[0])
+        for (int l = 0; l < nlev; ++l) {
+            const int D[3] = {(int)v->lay.level_dims[l][0], (int)v->lay.level_dims[l][1], (int)v->lay.level_dims[l][2]};
+            CK(v, launch_gather_quads(b.gq[l], b.dlev[l], D, l == 0, v->stream));
+            v->stats.launches += 1;
+        }
     if (lod && dvoxel_dev) {
         // each level's gradient onto the level it was filtered from, coarsest first (Sec. III-D)
         for (int l = v->L - 1; l >= 1; --l) {
