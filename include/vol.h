@@ -401,7 +401,10 @@ int vol_poll_requests(vol_t v, int32_t *out, int cap, int *n);
  * filter of level l-1 (Sec. III-D): their gradients are carried down to level
  * 0 through the filter's adjoint, 1/8 to each child (a child index past an
  * odd edge counts as the last voxel, as in the filter; integer storage is
- * differentiated as the mean).  Errors: VOL_ERR_NO_FORWARD_STATE (no gradient
+ * differentiated as the mean).  Its workspaces (sums of dL/dtf, up to 60 MB, and
+ * 16 bytes per voxel of the sampled levels when the rays' samples outnumber the
+ * voxels and the memory can be had) are taken by the gradient-mode vol_render and
+ * kept.  Errors: VOL_ERR_NO_FORWARD_STATE (no gradient
  * render, an incomplete one, or a level evicted since), VOL_ERR_INVALID_ARG
  * (NULL drgba_dev), VOL_ERR_CUDA. */
 int vol_render_backward(vol_t v, const float *drgba_dev, float *dtf_dev, float *dvoxel_dev);

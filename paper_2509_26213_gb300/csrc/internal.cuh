@@ -177,13 +177,15 @@ struct BackwardDev {
     int tile_w, tile_h;
     const float4* tf;
     float step;
+    float neg_zero;     // -0.0f, as in RenderDev
     float4 bg;
     const float4* drgba;
     float* dtf;
     float* dvox;                // level-0 gradient (NULL: none)
     float* dlev[kMaxLevels];    // gradient of each level's voxels; dlev[0] = dvox
     float4* gq[kMaxLevels];     // gradient quads of each level (gq[0] NULL: add to dlev directly)
-    float4* dtf_tabs;           // 256 entries per warp of the grid, zeroed
+    float4* dtf_tabs;           // dtf_copies tables of 256 entries per warp of the grid, zeroed
+    int dtf_copies;             // a power of two
     int lod_mode, lod_bias;
     unsigned* counters;
     const float* ckpt;
@@ -231,7 +233,7 @@ cudaError_t launch_gather_quads(const float4* gq, float* dvox, const int D[3], b
 // dtf += the sum of n 256-entry tables.
 cudaError_t launch_sum_tables(const float4* tabs, int n, float* dtf, cudaStream_t s);
 int backward_warps_per_cta();
-int backward_blocks_per_sm(int dtype, bool lod, bool tape);
+int backward_blocks_per_sm();
 
 // ---- launchers (kernels_volume.cu) ----
 // Each of these fills whole slots: the voxels, range[slot] = (min, max) of the stored values and

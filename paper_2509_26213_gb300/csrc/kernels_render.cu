@@ -13,22 +13,21 @@ __device__ __forceinline__ void red4(float4* p, float a, float b, float c, float
     asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d));
 }
 
-// dL/dtf accumulates in one 256-entry table per warp in global memory (L2), an entry's 4 channels by
-// one 16-byte reduction; k_sum_tables adds the tables up.  (Floating-point additions in shared
+// dL/dtf accumulates in 256-entry tables, one or more per warp, in global memory (L2), an entry's 4
+// channels by one 16-byte reduction; k_sum_tables adds the tables up.  (Floating-point additions in shared
 // memory are compare-and-swap loops, four of them per entry.)  Measured with the gradient quads
 // below and the segment's values kept in shared memory, 256^3, 16 views of 512x512: the adjoint
-// 7.93 -> 4.25 ms; 101x90x77 with 3 levels, 3 views of 203x151: 0.55 -> 0.26 ms.
-__device__ __forceinline__ void flush_dtf4(float4* tab, int idx, const float* acc) {
-    if (acc[0] != 0.0f || acc[1] != 0.0f || acc[2] != 0.0f || acc[3] != 0.0f)
-        red4(tab + idx, acc[0], acc[1], acc[2], acc[3]);
+// 7.0 -> 4.25 ms (with the pairs of the reverse sweep 3.72); 101x90x77 with 3 levels, 3 views of 203x151: 0.55 -> 0.26 ms.
+__device__ __forceinline__ void flush_dtf4(float4* tab, int idx, float2 rg, float2 ba) {
+    if (rg.x != 0.0f || rg.y != 0.0f || ba.x != 0.0f || ba.y != 0.0f) red4(tab + idx, rg.x, rg.y, ba.x, ba.y);
 }
-__device__ __forceinline__ void flush_dtf(float4* tab, int idx, float acc[8]) {
+__device__ __forceinline__ void flush_dtf(float4* tab, int idx, float2 acc[4]) {
     if (idx >= 0) {
-        flush_dtf4(tab, idx, acc);
-        flush_dtf4(tab, idx + 1, acc + 4);
+        flush_dtf4(tab, idx, acc[0], acc[1]);
+        flush_dtf4(tab, idx + 1, acc[2], acc[3]);
     }
 #pragma unroll
-    for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
+    for (int c = 0; c < 4; ++c) acc[c] = f2(0.0f);
 }
 
 // Adds the corner accumulators of trilinear cell `cell` to the level's gradient quads: entry
@@ -36,27 +35,27 @@ __device__ __forceinline__ void flush_dtf(float4* tab, int idx, float acc[8]) {
 // cell is two 16-byte reductions, at its lower corner's entry and the one a slice above (a slice of
 // padding takes those past the last).  Corners past an edge have weight 0.  k_gather_quads adds
 // the quads up per voxel.
-__device__ __forceinline__ void flush_quad(float4* gq, long long cell, long long slice, float cacc[8]) {
+__device__ __forceinline__ void flush_quad(float4* gq, long long cell, long long slice, float2 cacc[4]) {
     if (cell >= 0) {
-        red4(gq + cell, cacc[0], cacc[1], cacc[2], cacc[3]);
-        red4(gq + cell + slice, cacc[4], cacc[5], cacc[6], cacc[7]);
+        red4(gq + cell, cacc[0].x, cacc[0].y, cacc[1].x, cacc[1].y);
+        red4(gq + cell + slice, cacc[2].x, cacc[2].y, cacc[3].x, cacc[3].y);
     }
 #pragma unroll
-    for (int c = 0; c < 8; ++c) cacc[c] = 0.0f;
+    for (int r = 0; r < 4; ++r) cacc[r] = f2(0.0f);
 }
 
 // Adds the corner accumulators of trilinear cell `cell` (linear index of its lower corner;
-// cacc[cx + 2 cy + 4 cz]; mask: which +1 corners exist) to dvox, row by row (x-neighbour
+// cacc[cy + 2 cz] holds the corners at x and x + 1; mask: which +1 corners exist) to dvox, row by row (x-neighbour
 // pairs), skipping rows that do not exist or hold only zeros.  (16-byte vector atomics for the
 // pairs measured 2% slower than these scalar ones on the 16 x 512^2 workload.)
-__device__ __forceinline__ void flush_vox(float* dvox, long long cell, int mask, int Dx, int Dy, float cacc[8]) {
+__device__ __forceinline__ void flush_vox(float* dvox, long long cell, int mask, int Dx, int Dy, float2 cacc[4]) {
     if (cell >= 0) {
         const long long sy = Dx, sz = (long long)Dx * Dy;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int cy = r & 1, cz = r >> 1;
             const bool row_ok = (!cy || (mask & 2)) && (!cz || (mask & 4));
-            const float v0 = cacc[2 * r], v1 = (mask & 1) ? cacc[2 * r + 1] : 0.0f;
+            const float v0 = cacc[r].x, v1 = (mask & 1) ? cacc[r].y : 0.0f;
             if (!row_ok || (v0 == 0.0f && v1 == 0.0f)) continue;
             const long long L = cell + cy * sy + cz * sz;
             if (v0 != 0.0f) atomicAdd(dvox + L, v0);
@@ -64,7 +63,7 @@ __device__ __forceinline__ void flush_vox(float* dvox, long long cell, int mask,
         }
     }
 #pragma unroll
-    for (int c = 0; c < 8; ++c) cacc[c] = 0.0f;
+    for (int r = 0; r < 4; ++r) cacc[r] = f2(0.0f);
 }
 
 // Samples per lane whose page-table lookups and gathers the adjoint's forward recompute issues
@@ -75,14 +74,11 @@ __device__ __forceinline__ void flush_vox(float* dvox, long long cell, int mask,
 constexpr int kBwdBatch = VOLRC_BWD_BATCH;
 // Adjoint CTA size and the resident CTAs per SM its register allocation must allow (shared
 // memory per CTA: 4 KiB + 256 B per thread).
-#ifndef VOLRC_BWD_THREADS
-#define VOLRC_BWD_THREADS 192
-#endif
-#ifndef VOLRC_BWD_MINB
-#define VOLRC_BWD_MINB 4
-#endif
-constexpr int kBwdThreads = VOLRC_BWD_THREADS;
-constexpr int kBwdMinBlocks = VOLRC_BWD_MINB;
+// 160 threads: 49 KiB and up to 102 registers; 192 threads (57 KiB, 80 registers) leave the L1 next to
+// nothing and spill (16 views of 512x512, 256^3: forward + adjoint 7.72 against 7.97 ms; 128 threads at
+// 6 CTAs 8.30).
+constexpr int kBwdThreads = 160;
+constexpr int kBwdMinBlocks = 4;
 
 // Adjoint, warp-synchronous by checkpoint segment: a warp takes 32 rays (a ray tile, or a
 // 32-pixel part of it) and, round by round, processes segment s of every one of them that has
@@ -100,12 +96,18 @@ constexpr int kBwdMinBlocks = VOLRC_BWD_MINB;
 template <int DT, bool LOD, bool TAPE>
 __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_backward(const __grid_constant__ BackwardDev P) {
     __shared__ float4 s_tf[256];
-    // the warp's dL/dtf table
-    float4* const w_dtf = P.dtf_tabs + ((long long)blockIdx.x * (kBwdThreads / 32) + (threadIdx.x >> 5)) * 256;
+    __shared__ float4 s_tfd[255];  // tf[i+1] - tf[i], each difference rounded once
+    // the lane's dL/dtf table: lane l adds to copy l mod dtf_copies of its warp's
+    float4* const w_dtf = P.dtf_tabs + (((long long)blockIdx.x * (kBwdThreads / 32) + (threadIdx.x >> 5)) * P.dtf_copies +
+                                        ((int)threadIdx.x & (P.dtf_copies - 1))) * 256;
     __shared__ float s_T[kCkptEvery][kBwdThreads];
     __shared__ float s_V[kCkptEvery][kBwdThreads];  // (a lane's tape values are 128 B apart from its neighbour's: read once)
     __shared__ LevelDev s_lv[LOD ? kMaxLevels : 1];
     for (int i = threadIdx.x; i < 256; i += blockDim.x) s_tf[i] = P.tf[i];
+    for (int i = threadIdx.x; i < 255; i += blockDim.x) {
+        const float4 a = P.tf[i], b = P.tf[i + 1];
+        s_tfd[i] = make_float4(__fsub_rn(b.x, a.x), __fsub_rn(b.y, a.y), __fsub_rn(b.z, a.z), __fsub_rn(b.w, a.w));
+    }
     if (LOD && threadIdx.x < P.vol.nlevels) s_lv[threadIdx.x] = P.vol.lv[threadIdx.x];
     __syncthreads();
 
@@ -127,17 +129,17 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_backward(const _
     // per-lane accumulators: dL/dtf for entries acc_i, acc_i + 1; dL/dvoxel for the 8 corners
     // of cell cell_cur on level cell_lvl (cell_mask: which +1 corners exist)
     int acc_i = -1;
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float2 acc[4] = {f2(0.f), f2(0.f), f2(0.f), f2(0.f)};   // entry acc_i: red, green; blue, alpha; then acc_i + 1
     long long cell_cur = -1;
     int cell_mask = 0, cell_lvl = 0;
-    float cacc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float2 cacc[4] = {f2(0.f), f2(0.f), f2(0.f), f2(0.f)};  // corners (x, x + 1) of rows y + 2 z
 
     // lane state: the lane's ray, its sample count n and segment count nseg
     bool has = false;
     long long ray = 0;
     float o0 = 0, o1 = 0, o2 = 0, d0 = 0, d1 = 0, d2 = 0, t0 = 0, lodscale = 0;
     float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
-    float R0 = 0, R1 = 0, R2 = 0, R3 = 0;
+    float2 R01 = f2(0.f), R23 = f2(0.f);  // what lies behind the sample: colour, opacity
     int n = 0, nseg = 0;
     // warp-uniform: the segment index every lane processes in this round, descending; each
     // lane's rays sample the same depths as its neighbours' (adjacent pixels), so the gathers
@@ -174,7 +176,8 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_backward(const _
                     t0 = R.t0;
                     lodscale = V.lodscale;
                     g = P.drgba[ray];
-                    R0 = P.bg.x; R1 = P.bg.y; R2 = P.bg.z; R3 = P.bg.w;
+                    R01 = make_float2(P.bg.x, P.bg.y);
+                    R23 = make_float2(P.bg.z, P.bg.w);
                     nseg = ((n - 1) >> P.ckpt_shift) + 1;
                     has = true;
                 }
@@ -192,17 +195,22 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_backward(const _
         // the lane's segment on the tape: 32 values in 128 contiguous bytes
         const float* tp = TAPE ? P.tape + ((long long)s * P.nrays + (seg ? ray : 0)) * kCkptEvery : nullptr;
         if (TAPE) {
-            // forward from the tape, 4 values per load
-            for (int jb = 0; jb < maxlen; jb += 4) {
-                const float4 v4 = jb < len ? __ldg(reinterpret_cast<const float4*>(tp + jb)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float vv[4] = {v4.x, v4.y, v4.z, v4.w};
+            // forward from the tape, a 32-byte sector at a time (the lanes' values lie 128 bytes apart)
+            constexpr int TW = 8;
+            for (int jb = 0; jb < maxlen; jb += TW) {
+                float vv[TW];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
+                for (int q = 0; q < TW; q += 4) {
+                    const float4 v4 = jb + q < len ? __ldg(reinterpret_cast<const float4*>(tp + jb + q)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    vv[q] = v4.x, vv[q + 1] = v4.y, vv[q + 2] = v4.z, vv[q + 3] = v4.w;
+                }
+#pragma unroll
+                for (int u = 0; u < TW; ++u) {
                     if (jb + u < len) {
-                        const float x = tf_coord<DT>(vv[u]);
-                        const int i = min((int)x, 254);
-                        const float wt = x - (float)i;
-                        const float al = fmaf(wt, s_tf[i + 1].w - s_tf[i].w, s_tf[i].w);
+                        int i;
+                        float wt;
+                        tf_index<DT>(vv[u], i, wt);
+                        const float al = fmaf(wt, s_tfd[i].w, s_tf[i].w);
                         s_T[jb + u][tid] = T;
                         s_V[jb + u][tid] = vv[u];
                         T = T * (1.0f - al);
@@ -250,10 +258,10 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_backward(const _
             for (int u = 0; u < kBwdBatch; ++u) {
                 if (jb + u < len) {
                     if (slot[u] == kInvalidSlot) atomicAdd(&P.counters[kDevError], 1u);
-                    const float x = tf_coord<DT>(val[u]);
-                    const int i = min((int)x, 254);
-                    const float wt = x - (float)i;
-                    const float al = fmaf(wt, s_tf[i + 1].w - s_tf[i].w, s_tf[i].w);
+                    int i;
+                    float wt;
+                    tf_index<DT>(val[u], i, wt);
+                    const float al = fmaf(wt, s_tfd[i].w, s_tf[i].w);
                     s_T[jb + u][tid] = T;
                     s_V[jb + u][tid] = val[u];
                     T = T * (1.0f - al);
@@ -263,11 +271,13 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_backward(const _
         float kf = (float)(k0 + maxlen - 1);  // (float)(k0 + j), stepped down exactly
         for (int j = maxlen - 1; j >= 0; --j, kf = __fsub_rn(kf, 1.0f)) {
             if (j < len) {
-                Resolved Q;  // the sample's voxel and weights: only dL/dvoxel needs them
+                // (the arithmetic goes by packed pairs: channels, axes x and y, corners x and x + 1;
+                // the kernel is bound by instruction issue)
+                float2 w01 = f2(0.f);  // the sample's weights and voxel: only dL/dvoxel needs them
+                float w2 = 0.f;
+                int i0 = 0, i1 = 0, i2 = 0;
                 if (P.dvox) {
                     const float t = __fadd_rn(t0, __fmul_rn(kf, step));
-                    const float p[3] = {__fadd_rn(o0, __fmul_rn(t, d0)), __fadd_rn(o1, __fmul_rn(t, d1)),
-                                        __fadd_rn(o2, __fmul_rn(t, d2))};
                     if (LOD) {
                         const int l = lod_level(t, lodscale, P.lod_bias, nlev);
                         if (l != cur_l) {
@@ -275,60 +285,76 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_backward(const _
                             L0 = load_lv(s_lv[l]);
                         }
                     }
-                    resolve_reg(L0, bshift, bmask, row, p, Q);
+                    // resolve_reg's positions and clamp (level 0: the ratio is exactly 1)
+                    const float nz = P.neg_zero;
+                    float2 x01 = add2(make_float2(o0, o1), mul2(f2(t), make_float2(d0, d1), nz));
+                    float x2 = __fadd_rn(o2, __fmul_rn(t, d2));
+                    if (LOD) {
+                        x01 = mul2(x01, make_float2(L0.r[0], L0.r[1]), nz);
+                        x2 = __fmul_rn(x2, L0.r[2]);
+                    }
+                    x01 = add2(x01, f2(-0.5f));
+                    x2 = __fsub_rn(x2, 0.5f);
+                    x01 = make_float2(fminf(fmaxf(x01.x, 0.0f), L0.Dm[0]), fminf(fmaxf(x01.y, 0.0f), L0.Dm[1]));
+                    x2 = fminf(fmaxf(x2, 0.0f), L0.Dm[2]);
+                    const float2 fl01 = make_float2(floorf(x01.x), floorf(x01.y));
+                    const float fl2 = floorf(x2);
+                    w01 = fma2(fl01, f2(-1.0f), x01);
+                    w2 = __fsub_rn(x2, fl2);
+                    i0 = (int)fl01.x;
+                    i1 = (int)fl01.y;
+                    i2 = (int)fl2;
                 }
                 const float val = s_V[j][tid];
                 const float Tk = s_T[j][tid];
-                const float x = tf_coord<DT>(val);
-                const int i = min((int)x, 254);
-                const float wt = x - (float)i;
-                const float4 a = s_tf[i], b = s_tf[i + 1];
-                const float cr = fmaf(wt, b.x - a.x, a.x), cg = fmaf(wt, b.y - a.y, a.y);
-                const float cb = fmaf(wt, b.z - a.z, a.z), al = fmaf(wt, b.w - a.w, a.w);
-                const float dal = Tk * (g.x * (cr - R0) + g.y * (cg - R1) + g.z * (cb - R2) + g.w * (1.0f - R3));
+                int i;
+                float wt;
+                tf_index<DT>(val, i, wt);
+                const float4 a = s_tf[i], b = s_tfd[i];
+                const float2 b01 = make_float2(b.x, b.y), b23 = make_float2(b.z, b.w);
+                const float2 c01 = fma2(f2(wt), b01, make_float2(a.x, a.y)), c23 = fma2(f2(wt), b23, make_float2(a.z, a.w));
+                const float al = c23.y;
+                const float2 e01 = fma2(R01, f2(-1.0f), c01), e23 = fma2(R23, f2(-1.0f), make_float2(c23.x, 1.0f));
+                const float2 g01 = make_float2(g.x, g.y), g23 = make_float2(g.z, g.w);
+                const float2 ge = fma2(g01, e01, fma2(g23, e23, f2(0.0f)));
+                const float dal = Tk * (ge.x + ge.y);
                 const float Ta = Tk * al;
-                const float dr = g.x * Ta, dg = g.y * Ta, db = g.z * Ta;
+                const float2 q01 = fma2(g01, f2(Ta), f2(0.0f));         // dL/d(red, green) of the row
+                const float2 q23 = make_float2(g.z * Ta, dal);          // blue, alpha
+                R01 = fma2(f2(al), e01, R01);
+                R23 = fma2(f2(al), e23, R23);
                 if (P.dtf) {
                     // register accumulation while the TF index stays the same
                     if (i != acc_i) {
                         // to a neighbouring index the entry both lookups share stays in registers:
                         // only the one left behind is added to the table
-                        if (acc_i >= 0 && i == acc_i + 1) {
-                            flush_dtf4(w_dtf, acc_i, acc);
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                acc[c] = acc[4 + c];
-                                acc[4 + c] = 0.0f;
-                            }
-                        } else if (acc_i >= 0 && i == acc_i - 1) {
-                            flush_dtf4(w_dtf, acc_i + 1, acc + 4);
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                acc[4 + c] = acc[c];
-                                acc[c] = 0.0f;
-                            }
+                        const bool up = i == acc_i + 1, down = i == acc_i - 1;
+                        if (acc_i >= 0 && (up || down)) {
+                            flush_dtf4(w_dtf, up ? acc_i : acc_i + 1, up ? acc[0] : acc[2], up ? acc[1] : acc[3]);
+                            const float2 k0 = up ? acc[2] : acc[0], k1 = up ? acc[3] : acc[1];
+                            acc[0] = up ? k0 : f2(0.0f);
+                            acc[1] = up ? k1 : f2(0.0f);
+                            acc[2] = up ? f2(0.0f) : k0;
+                            acc[3] = up ? f2(0.0f) : k1;
                         } else {
                             flush_dtf(w_dtf, acc_i, acc);
                         }
                         acc_i = i;
                     }
                     const float w0 = 1.0f - wt;
-                    acc[0] = fmaf(w0, dr, acc[0]);
-                    acc[1] = fmaf(w0, dg, acc[1]);
-                    acc[2] = fmaf(w0, db, acc[2]);
-                    acc[3] = fmaf(w0, dal, acc[3]);
-                    acc[4] = fmaf(wt, dr, acc[4]);
-                    acc[5] = fmaf(wt, dg, acc[5]);
-                    acc[6] = fmaf(wt, db, acc[6]);
-                    acc[7] = fmaf(wt, dal, acc[7]);
+                    acc[0] = fma2(f2(w0), q01, acc[0]);
+                    acc[1] = fma2(f2(w0), q23, acc[1]);
+                    acc[2] = fma2(f2(wt), q01, acc[2]);
+                    acc[3] = fma2(f2(wt), q23, acc[3]);
                 }
                 if (P.dvox && tf_inside<DT>(val)) {
-                    const float dv = 255.0f * (dr * (b.x - a.x) + dg * (b.y - a.y) + db * (b.z - a.z) + dal * (b.w - a.w));
+                    const float2 qb = fma2(q01, b01, fma2(q23, b23, f2(0.0f)));
+                    const float dv = 255.0f * (qb.x + qb.y);
                     if (dv != 0.0f) {
                         // register accumulation while the trilinear cell (and level) stays the same
                         const int lq = LOD ? cur_l : 0;
                         const int Dx = (int)L0.Dm[0] + 1, Dy = (int)L0.Dm[1] + 1;
-                        const long long cell = (long long)Q.i0[0] + (long long)Dx * ((long long)Q.i0[1] + (long long)Dy * Q.i0[2]);
+                        const long long cell = (long long)i0 + (long long)Dx * ((long long)i1 + (long long)Dy * i2);
                         if (cell != cell_cur || lq != cell_lvl) {
                             if (P.gq[0])
                                 flush_quad(P.gq[cell_lvl], cell_cur, (long long)dim_x(cell_lvl) * dim_y(cell_lvl), cacc);
@@ -336,22 +362,17 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_backward(const _
                                 flush_vox(P.dlev[cell_lvl], cell_cur, cell_mask, dim_x(cell_lvl), dim_y(cell_lvl), cacc);
                             cell_cur = cell;
                             cell_lvl = lq;
-                            cell_mask = ((float)Q.i0[0] < L0.Dm[0] ? 1 : 0) | ((float)Q.i0[1] < L0.Dm[1] ? 2 : 0) |
-                                        ((float)Q.i0[2] < L0.Dm[2] ? 4 : 0);
+                            cell_mask = ((float)i0 < L0.Dm[0] ? 1 : 0) | ((float)i1 < L0.Dm[1] ? 2 : 0) |
+                                        ((float)i2 < L0.Dm[2] ? 4 : 0);
                         }
-                        const float wx = Q.w[0], wy = Q.w[1], wz = Q.w[2];
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;
-                            const float wgt = (cx ? wx : 1.0f - wx) * (cy ? wy : 1.0f - wy) * (cz ? wz : 1.0f - wz);
-                            cacc[c] = fmaf(wgt, dv, cacc[c]);
-                        }
+                        const float2 wx = make_float2(1.0f - w01.x, w01.x);
+                        const float v0 = (1.0f - w2) * dv, v1 = w2 * dv, wy0 = 1.0f - w01.y;
+                        cacc[0] = fma2(wx, f2(wy0 * v0), cacc[0]);
+                        cacc[1] = fma2(wx, f2(w01.y * v0), cacc[1]);
+                        cacc[2] = fma2(wx, f2(wy0 * v1), cacc[2]);
+                        cacc[3] = fma2(wx, f2(w01.y * v1), cacc[3]);
                     }
                 }
-                R0 = fmaf(al, cr - R0, R0);
-                R1 = fmaf(al, cg - R1, R1);
-                R2 = fmaf(al, cb - R2, R2);
-                R3 = fmaf(al, 1.0f - R3, R3);
             }
         }
         --s;
@@ -363,29 +384,28 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_backward(const _
     }
 }
 
-// dtf[entry] += the sum of that entry over the warps' tables, in binary64 (one CTA per entry).
-constexpr int kSumThreads = 256;
+// dtf[entry] += the sums of the entries over the tables: a CTA takes 8 entries (a 128-byte line of
+// every table) of one in kSumSlices slices of the tables and sums them in binary64.
+constexpr int kSumThreads = 256, kSumSlices = 16;
 
-__global__ void __launch_bounds__(kSumThreads) k_sum_tables(const float4* __restrict__ tabs, int n, float4* dtf) {
-    __shared__ double s_sum[kSumThreads / 32][4];
+__global__ void __launch_bounds__(kSumThreads) k_sum_tables(const float4* __restrict__ tabs, int n, float* dtf) {
+    __shared__ double s_sum[kSumThreads / 8][8][4];
+    const int q = threadIdx.x & 7, r = threadIdx.x >> 3;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int t = threadIdx.x; t < n; t += kSumThreads) {
-        const float4 a = tabs[(long long)t * 256 + blockIdx.x];
+    for (int t = (int)blockIdx.y * (kSumThreads / 8) + r; t < n; t += kSumSlices * (kSumThreads / 8)) {
+        const float4 a = tabs[(long long)t * 256 + blockIdx.x * 8 + q];
         v[0] += a.x;
         v[1] += a.y;
         v[2] += a.z;
         v[3] += a.w;
     }
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        for (int o = 16; o; o >>= 1) v[c] += __shfl_xor_sync(kFull, v[c], o);
-        if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5][c] = v[c];
-    }
+    for (int c = 0; c < 4; ++c) s_sum[r][q][c] = v[c];
     __syncthreads();
-    if (threadIdx.x < 4) {
+    if (threadIdx.x < 32) {
         double sum = 0.0;
-        for (int w = 0; w < kSumThreads / 32; ++w) sum += s_sum[w][threadIdx.x];
-        ((float*)(dtf + blockIdx.x))[threadIdx.x] += (float)sum;
+        for (int w = 0; w < kSumThreads / 8; ++w) sum += s_sum[w][threadIdx.x >> 2][threadIdx.x & 3];
+        if (sum != 0.0) atomicAdd(dtf + blockIdx.x * 32 + threadIdx.x, (float)sum);
     }
 }
 
@@ -609,7 +629,7 @@ cudaError_t launch_backward(int dtype, const BackwardDev& p, int grid, cudaStrea
 }
 
 cudaError_t launch_sum_tables(const float4* tabs, int n, float* dtf, cudaStream_t s) {
-    k_sum_tables<<<256, kSumThreads, 0, s>>>(tabs, n, (float4*)dtf);
+    k_sum_tables<<<dim3(32, kSumSlices), kSumThreads, 0, s>>>(tabs, n, dtf);
     return cudaGetLastError();
 }
 
@@ -642,11 +662,7 @@ cudaError_t launch_trace(const TraceDev& p, cudaStream_t s) {
 
 int backward_warps_per_cta() { return kBwdThreads / 32; }
 
-int backward_blocks_per_sm(int dtype, bool lod, bool tape) {
-    int n = 0;
-    const void* fn = pick_backward(dtype, lod, tape);
-    if (!fn || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kBwdThreads, 0) != cudaSuccess) return 1;
-    return n > 0 ? n : 1;
-}
+// (what the launch bounds allot registers for; the shared memory allows 4 as well)
+int backward_blocks_per_sm() { return kBwdMinBlocks; }
 
 }  // namespace volrc

@@ -202,11 +202,13 @@ struct SlotSource {
 // a cell are reduced by shuffles at the end.  The rows and slices that two cells share are read
 // again, from L1 or L2.
 // WRITE: store the words; MS: log2 M.
-// 512 threads at 2 CTAs per SM (64 registers): one CTA per SM with all a slice's words in registers
-// is slower (512^3 u16 update, 32^3 bricks: 1.10 against 1.02 ms), 256-thread CTAs too.
-// Measured, 512^3 u16 into quad slots (0.27 GB read, 1.07 GB written): 258 us; its first coarser
-// level 128 us, the small ones 25 us.  With upload, filter and ranges as separate passes and a slot
-// list allocated per call, a time step (upload, pyramid, 1280x720 frame) took 3.30 ms; now 0.84.
+// Uploads: 512 threads at 2 CTAs per SM (64 registers); one CTA per SM is slower (512^3 u16 update,
+// 32^3 bricks: 1.10 against 1.02 ms), 256-thread CTAs too.  The filter holds 8 words per voxel of a
+// slice and takes one CTA per SM: at 64 registers its small levels, where latency counts, take 34
+// to 52 us instead of 25 to 40, the large one as long.
+// Measured, 512^3 u16 into quad slots (0.27 GB read, 1.07 GB written): 1033 (upload) + 708 (ranges)
+// -> 257 us; its first coarser level 627 + 138 -> 125 us; a time step (upload, pyramid, 1280x720
+// frame) with a slot list allocated per call 3.30 -> 0.84 ms.
 constexpr int kFillThreads = 512;
 
 template <int DT, int MS, bool WRITE, class Source>
@@ -332,7 +334,7 @@ __global__ void __launch_bounds__(kFillThreads, 2) k_upload_level(const typename
 }
 
 template <int DT, int MS, bool Q>
-__global__ void __launch_bounds__(kFillThreads, 2) k_downsample(typename Stored<DT>::T* atlas, const __grid_constant__ VolDev vol,
+__global__ void __launch_bounds__(kFillThreads, 1) k_downsample(typename Stored<DT>::T* atlas, const __grid_constant__ VolDev vol,
                                                              int level, float2* range, uint16_t* cells,
                                                              const uint32_t* __restrict__ slots, long long nbricks, unsigned* err) {
     const LevelDev &L = vol.lv[level], &F = vol.lv[level - 1];

@@ -949,8 +949,9 @@ template <int DT>
 __device__ __forceinline__ void tf_index(float val, int& i, float& wt) {
     const float u = tf_unscaled<DT>(val);
     const float x = DT == VOL_U8 ? u : __fmul_rn(u, tf_scale<DT>);
-    i = min((int)x, 254);
-    wt = __fsub_rn(x, (float)i);
+    const float m = fminf(__fadd_rd(x, 8388608.0f), 8388608.0f + 254.0f);  // 2^23 + i (batch_positions)
+    i = (int)(__float_as_uint(m) & 255u);
+    wt = __fsub_rn(x, __fsub_rn(m, 8388608.0f));
 }
 // The same for two samples (floor by 2^23 as in batch_positions; x lies in [0, 255]).
 template <int DT>

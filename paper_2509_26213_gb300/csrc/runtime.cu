@@ -610,6 +610,34 @@ int ensure_miss_buffers(vol_t v) {
     return VOL_OK;
 }
 
+// Gradient quads for the adjoint of the current views (levels 0 .. L-1 with LOD).  They cost 16 B of
+// zeroing, 16 B of reading and the voxel's own update per voxel, and save 6 of 8 reductions per cell
+// visit: taken when the rays' samples (about an eighth of pixels x longest axis / step in the
+// measured frames) outnumber the voxels, and the memory can be had.
+bool ensure_quads(vol_t v, bool lod) {
+    size_t quads = 0, voxels = 0;
+    for (int l = 0; l < (lod ? v->L : 1); ++l) {
+        const int64_t* D = v->lay.level_dims[l];
+        voxels += (size_t)(D[0] * D[1] * D[2]);
+        quads += (size_t)(D[0] * D[1] * (D[2] + 1));
+    }
+    const double longest = (double)std::max({v->lay.dims[0], v->lay.dims[1], v->lay.dims[2]});
+    if ((double)v->nrays * longest / (double)v->params.step < 8.0 * (double)voxels) return false;
+    if (ensure(v, v->gq_buf, v->gq_cap, quads, "gradient quads") == VOL_OK) return true;
+    cudaGetLastError();  // (the failed allocation: the gradients go to the voxels directly)
+    v->err.clear();
+    return false;
+}
+
+// The adjoint's dL/dtf tables: copies per warp, and the entries of all of them.  4 tables per warp
+// where a warp takes many rays: a quarter of the additions to each, and half of their rounding; for
+// few rays the tables' zeroing and summing would show.
+int ensure_tables(vol_t v, int* copies, size_t* entries) {
+    *copies = v->nrays >= (1 << 20) ? 4 : 1;
+    *entries = (size_t)backward_blocks_per_sm() * v->nsm * backward_warps_per_cta() * *copies * 256;
+    return ensure(v, v->dtf_tabs, v->dtf_tabs_cap, *entries, "dL/dtf tables");
+}
+
 RenderDev render_args(vol_t v) {
     RenderDev p{};
     p.vol = vol_dev(v);
@@ -1730,6 +1758,11 @@ int vol_render(vol_t v, const vol_camera* cams, int nviews, const float* tf_dev,
                 v->err.clear();
             }
         }
+        // the adjoint's workspaces too, so that it allocates nothing (it can be captured)
+        int copies;
+        size_t entries;
+        if (int rc = ensure_tables(v, &copies, &entries)) return rc;
+        ensure_quads(v, p.lod_mode != 0);
     }
     // scheduling state: the previous frame's longest-ray-first order is reused while the tile
     // partition (tile shape, number of views, image sizes) is unchanged; cameras may move.
@@ -1821,6 +1854,7 @@ int vol_render_backward(vol_t v, const float* drgba_dev, float* dtf_dev, float* 
         return fail(v, VOL_ERR_NO_FORWARD_STATE, lod ? "a level is no longer fully resident" : "level 0 changed since the render");
     if (!dtf_dev && !dvoxel_dev) return VOL_OK;
     BackwardDev b{};
+    b.neg_zero = -0.0f;
     b.vol = vol_dev(v);
     b.views = v->views_dev;
     b.nviews = v->nviews;
@@ -1850,29 +1884,13 @@ int vol_render_backward(vol_t v, const float* drgba_dev, float* dtf_dev, float* 
     }
     const int nlev = lod ? v->L : 1;
     if (dvoxel_dev) {
-        // Gradient quads cost 16 B of zeroing, 16 B of reading and the voxel's own update per voxel,
-        // and save 6 of 8 reductions per cell visit: taken when the rays' samples (about an eighth of
-        // pixels x longest axis / step in the measured frames) outnumber the voxels, and the memory
-        // can be had.
-        size_t quads = 0, voxels = 0;
-        for (int l = 0; l < nlev; ++l) {
-            const int64_t* D = v->lay.level_dims[l];
-            voxels += (size_t)(D[0] * D[1] * D[2]);
-            quads += (size_t)(D[0] * D[1] * (D[2] + 1));
-        }
-        const double longest = (double)std::max({v->lay.dims[0], v->lay.dims[1], v->lay.dims[2]});
-        if ((double)v->nrays * longest / (double)v->params.step >= 8.0 * (double)voxels) {
-            if (ensure(v, v->gq_buf, v->gq_cap, quads, "gradient quads") == VOL_OK) {
-                CK(v, cudaMemsetAsync(v->gq_buf, 0, sizeof(float4) * quads, v->stream));
-                size_t off = 0;
-                for (int l = 0; l < nlev; ++l) {
-                    b.gq[l] = v->gq_buf + off;
-                    off += (size_t)(v->lay.level_dims[l][0] * v->lay.level_dims[l][1] * (v->lay.level_dims[l][2] + 1));
-                }
-            } else {
-                cudaGetLastError();  // (the failed allocation: the gradients go to the voxels directly)
-                v->err.clear();
+        if (ensure_quads(v, lod)) {
+            size_t off = 0;
+            for (int l = 0; l < nlev; ++l) {
+                b.gq[l] = v->gq_buf + off;
+                off += (size_t)(v->lay.level_dims[l][0] * v->lay.level_dims[l][1] * (v->lay.level_dims[l][2] + 1));
             }
+            CK(v, cudaMemsetAsync(v->gq_buf, 0, sizeof(float4) * off, v->stream));
         }
         if (lod && !b.gq[0]) {
             size_t tot = 0;
@@ -1892,17 +1910,17 @@ int vol_render_backward(vol_t v, const float* drgba_dev, float* dtf_dev, float* 
     CK(v, cudaMemsetAsync(v->counters, 0, sizeof(unsigned) * kNumCounters, v->stream));
     v->counters_collected = false;  // vol_get_stats adds the adjoint's device-side check count
     v->last_counters = v->counters;
-    const int grid = backward_blocks_per_sm(v->dtype, lod, b.tape != nullptr) * v->nsm;
+    const int grid = backward_blocks_per_sm() * v->nsm;
     if (dtf_dev) {
-        const size_t n = (size_t)grid * backward_warps_per_cta() * 256;
-        if (int rc = ensure(v, v->dtf_tabs, v->dtf_tabs_cap, n, "dL/dtf tables")) return rc;
+        size_t n;
+        if (int rc = ensure_tables(v, &b.dtf_copies, &n)) return rc;
         CK(v, cudaMemsetAsync(v->dtf_tabs, 0, sizeof(float4) * n, v->stream));
         b.dtf_tabs = v->dtf_tabs;
     }
     CK(v, launch_backward(v->dtype, b, grid, v->stream));
     v->stats.launches += 1;
     if (dtf_dev) {
-        CK(v, launch_sum_tables(v->dtf_tabs, grid * backward_warps_per_cta(), dtf_dev, v->stream));
+        CK(v, launch_sum_tables(v->dtf_tabs, grid * backward_warps_per_cta() * b.dtf_copies, dtf_dev, v->stream));
         v->stats.launches += 1;
     }
     if (b.gq[0])
